@@ -47,7 +47,7 @@ def source_digest(kernel: str = "linattn_fused_tc"):
     they were taken on."""
     import hashlib
     h = hashlib.sha256()
-    names = ["sm100_kernels.cuh", "sm100_ptx.cuh", "tensor_map.hpp"] + (["sm100_backward.cuh"] if "bwd" in kernel else [])
+    names = ["sm100_kernels.cuh", "sm100_ptx.cuh", "f32x2.cuh", "tensor_map.hpp"] + (["sm100_backward.cuh"] if "bwd" in kernel else [])
     for name in names:
         h.update(open(os.path.join(ROOT, "paper_2510_08318_b200", "csrc", name), "rb").read())
     return h.hexdigest()[:16]

@@ -196,17 +196,15 @@ void prof_mark(linattn_ctx* c, cudaStream_t st, const char* name, double alg_byt
     c->prof_pending = true;
 }
 
-// Splits of the token range per (b,h) for the key-side reduction: enough CTAs to fill the GPU,
-// never shorter than 256 tokens each; a function of (G, n) only, so results are reproducible.
-int choose_splits(long long G, int n, int forced)
+// Key-side partial reductions per (b,h) pair that LINATTN_OPT_SPLITS asks for, 0 = the kernels' own deal: at most one per
+// 32 tokens, none empty.
+int forced_splits(int n, int forced)
 {
-    long long s = forced > 0 ? forced : (kTargetCtas + G - 1) / G;
-    const long long by_len = (n + 255) / 256;
-    if (forced <= 0 && s > by_len) s = by_len;
-    if (s > n) s = n;
-    if (s > kMaxSplits) s = kMaxSplits;
-    if (s < 1) s = 1;
-    return (int)s;
+    if (forced <= 0) return 0;
+    long long s = forced < n ? forced : n;
+    long long chunk = (n + s - 1) / s;
+    chunk = (chunk + 31) / 32 * 32;
+    return (int)((n + chunk - 1) / chunk);
 }
 
 template <typename T, int D>
@@ -218,37 +216,24 @@ linattn_status launch_simt(linattn_ctx* c, const void* q, const void* k, const v
     const float* Wq = c->Wq + (size_t)c->view_head0 * D * (D / 2);
     const float* Wk = c->Wk + (size_t)c->view_head0 * D * (D / 2);
     float* state = c->state + (size_t)c->view_g0 * (D * D + D);
-    int splits = choose_splits(G, n, c->opt_splits);
-    // token chunk per split, rounded up to the kernel's 32-token step; drop splits left empty
-    int chunk = (n + splits - 1) / splits;
-    chunk = (chunk + kSimtTokens - 1) / kSimtTokens * kSimtTokens;
-    splits = (n + chunk - 1) / chunk;
-    if (G * splits > c->partial_slots) return LINATTN_ERR_WORKSPACE;
-    constexpr int E = D * D + D;
+    const int forced = forced_splits(n, c->opt_splits);
+    if (G * forced > c->partial_slots) return LINATTN_ERR_WORKSPACE;
+    const SimtRuns rk = kside_runs<D>(G, n, forced), rq = qside_runs<D>(G, n);
 
     bool& attr_done = c->attr_done[linattn_ctx::kAttrSimtFwd + (sizeof(T) == 2 ? 2 : 0) + (D == 128 ? 1 : 0)];
     if (!attr_done) {
-        LA_CUDA(c, cudaFuncSetAttribute(kside_simt<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)kside_simt_smem<D>()));
-        LA_CUDA(c, cudaFuncSetAttribute(qside_simt<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)qside_simt_smem<D>()));
+        LA_CUDA(c, (simt_forward_attributes<T, D>()));
         attr_done = true;
     }
     const double side_bytes = 2.0 * (double)G * n * D * sizeof(T);  // K+V read, or Q read + O written
     prof_begin(c, st);
-    kside_simt<T, D><<<dim3(splits, (unsigned)G), kSimtThreads, kside_simt_smem<D>(), st>>>(
-        (const T*)k, (const T*)v, Wk, c->partial, Hv, n, chunk, act_strides(c, n), c->opt_phi);
+    launch_kside_simt<T, D>(rk, (const T*)k, (const T*)v, Wk, c->partial, Hv, n, act_strides(c, n), c->opt_phi, st);
     LA_CUDA(c, cudaGetLastError());
     prof_mark(c, st, "kside_simt", side_bytes);
-    combine_state<<<dim3((E + 255) / 256, (unsigned)G), 256, 0, st>>>(c->partial, state, splits, E);
+    launch_combine_state<D>(rk, c->partial, state, G, st);
     LA_CUDA(c, cudaGetLastError());
     prof_mark(c, st, "combine_state", 0.0);
-    const int nchunks = (n + kSimtTokens - 1) / kSimtTokens;
-    long long per_group = (2LL * 148 + G - 1) / G;
-    if (per_group > nchunks) per_group = nchunks;
-    if (per_group < 1) per_group = 1;
-    qside_simt<T, D><<<dim3((unsigned)per_group, (unsigned)G), kSimtThreads, qside_simt_smem<D>(), st>>>(
-        (const T*)q, Wq, state, (T*)out, Hv, n, (const T*)mix, mix_r, act_strides(c, n), c->opt_phi);
+    launch_qside_simt<T, D>(rq, (const T*)q, Wq, state, (T*)out, Hv, n, (const T*)mix, mix_r, act_strides(c, n), c->opt_phi, st);
     LA_CUDA(c, cudaGetLastError());
     prof_mark(c, st, "qside_simt", side_bytes);
     c->last_launches = 3;
@@ -271,19 +256,17 @@ linattn_status launch_backward_simt(linattn_ctx* c, const void* q, const void* k
                                     const MixGrad& mg)
 {
     const long long G = (long long)B * c->H;
-    int splits = choose_splits(G, n, c->opt_splits);
-    int chunk = (n + splits - 1) / splits;
-    chunk = (chunk + kSimtTokens - 1) / kSimtTokens * kSimtTokens;
-    splits = (n + chunk - 1) / chunk;
+    const int forced = forced_splits(n, c->opt_splits);
+    const SimtRuns rk = kside_runs<D>(G, n, forced);
     const int nchunks = (n + kSimtTokens - 1) / kSimtTokens;
     long long blocks = (kTargetCtas + G - 1) / G;   // blocks per (b,h) of the two gradient kernels
     if (blocks > nchunks) blocks = nchunks;
-    if (G * splits > c->partial_slots || G * blocks > c->partial_slots) return LINATTN_ERR_WORKSPACE;
+    if (G * forced > c->partial_slots || G * blocks > c->partial_slots) return LINATTN_ERR_WORKSPACE;
     constexpr int E = D * D + D, DM = D * (D / 2);
 
     bool& attr_done = c->attr_done[linattn_ctx::kAttrSimtBwd + (sizeof(T) == 2 ? 2 : 0) + (D == 128 ? 1 : 0)];
     if (!attr_done) {
-        LA_CUDA(c, cudaFuncSetAttribute(kside_simt<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kside_simt_smem<D>()));
+        LA_CUDA(c, (simt_forward_attributes<T, D>()));
         LA_CUDA(c, cudaFuncSetAttribute(qside_bwd<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bwd_smem<D>()));
         LA_CUDA(c, cudaFuncSetAttribute(kside_bwd<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bwd_smem<D>()));
         attr_done = true;
@@ -293,11 +276,10 @@ linattn_status launch_backward_simt(linattn_ctx* c, const void* q, const void* k
     const dim3 grid((unsigned)blocks, (unsigned)G);
     prof_begin(c, st);
     const int relu = c->opt_phi;
-    kside_simt<T, D><<<dim3(splits, (unsigned)G), kSimtThreads, kside_simt_smem<D>(), st>>>(
-        (const T*)k, (const T*)v, c->Wk, c->partial, c->H, n, chunk, as, relu);
+    launch_kside_simt<T, D>(rk, (const T*)k, (const T*)v, c->Wk, c->partial, c->H, n, as, relu, st);
     LA_CUDA(c, cudaGetLastError());
     prof_mark(c, st, "kside_simt", 2.0 * tensor_bytes);
-    combine_state<<<dim3((E + 255) / 256, (unsigned)G), 256, 0, st>>>(c->partial, c->state, splits, E);
+    launch_combine_state<D>(rk, c->partial, c->state, G, st);
     LA_CUDA(c, cudaGetLastError());
     prof_mark(c, st, "combine_state", 0.0);
     qside_bwd<T, D><<<grid, kSimtThreads, bwd_smem<D>(), st>>>((const T*)q, (const T*)dout, c->Wq, c->state, (T*)dq,
@@ -306,7 +288,7 @@ linattn_status launch_backward_simt(linattn_ctx* c, const void* q, const void* k
     LA_CUDA(c, cudaGetLastError());
     prof_mark(c, st, "qside_bwd", 3.0 * tensor_bytes);
     int launches = 5;
-    combine_state<<<dim3((E + 255) / 256, (unsigned)G), 256, 0, st>>>(c->bwd_part_state, c->bwd_dstate, (int)blocks, E);
+    combine_blocks<<<dim3((E + 255) / 256, (unsigned)G), 256, 0, st>>>(c->bwd_part_state, c->bwd_dstate, (int)blocks, E);
     LA_CUDA(c, cudaGetLastError());
     const dim3 wgrid((DM + 255) / 256, per_head ? (unsigned)c->H : 1u);
     if (!relu) {   // the ReLU kernel function has no weights

@@ -65,12 +65,8 @@ template <typename T, int D>
 linattn_status run(int dev, int slot, float* scratch, const T* q, const T* k, const T* v, T* out, const float* Wq,
                    const float* Wk, int Hw, long long G, int n, cudaStream_t st)
 {
-    constexpr int E = D * D + D;
     if (!g_attr_done[dev][slot]) {
-        if (cudaFuncSetAttribute(kside_simt<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kside_simt_smem<D>()) != cudaSuccess ||
-            cudaFuncSetAttribute(qside_simt<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)qside_simt_smem<D>()) != cudaSuccess) {
+        if (simt_forward_attributes<T, D>() != cudaSuccess) {
             cudaGetLastError();
             return LINATTN_ERR_CUDA;
         }
@@ -81,20 +77,14 @@ linattn_status run(int dev, int slot, float* scratch, const T* q, const T* k, co
     const long long by_len = ((long long)n + 255) / 256;
     if (splits > by_len) splits = by_len;
     if (splits < 1) splits = 1;
-    int chunk = (int)((n + splits - 1) / splits);
-    chunk = (chunk + kSimtTokens - 1) / kSimtTokens * kSimtTokens;
-    splits = (n + chunk - 1) / chunk;
 
-    float* partial = scratch;                                              // [G*splits][E], fully overwritten
+    float* partial = scratch;                                              // one record per CTA, every one that is read written first
     float* state = scratch + (size_t)kNoAllocPartialSlots * kNoAllocMaxE;  // [G][E], fully overwritten
-    kside_simt<T, D><<<dim3((unsigned)splits, (unsigned)G), kSimtThreads, kside_simt_smem<D>(), st>>>(
-        k, v, Wk, partial, Hw, n, chunk, ActStrides{D, (long long)n * D, (long long)Hw * n * D}, 0);
-    combine_state<<<dim3((E + 255) / 256, (unsigned)G), 256, 0, st>>>(partial, state, (int)splits, E);
-    const int nchunks = (n + kSimtTokens - 1) / kSimtTokens;
-    long long per_group = (2LL * 148 + G - 1) / G;
-    if (per_group > nchunks) per_group = nchunks;
-    qside_simt<T, D><<<dim3((unsigned)per_group, (unsigned)G), kSimtThreads, qside_simt_smem<D>(), st>>>(
-        q, Wq, state, out, Hw, n, (const T*)nullptr, 0.f, ActStrides{D, (long long)n * D, (long long)Hw * n * D}, 0);
+    const ActStrides as{D, (long long)n * D, (long long)Hw * n * D};
+    const SimtRuns r = kside_runs<D>(G, n, (int)splits);
+    launch_kside_simt<T, D>(r, k, v, Wk, partial, Hw, n, as, 0, st);
+    launch_combine_state<D>(r, partial, state, G, st);
+    launch_qside_simt<T, D>(qside_runs<D>(G, n), q, Wq, state, out, Hw, n, (const T*)nullptr, 0.f, as, 0, st);
     if (cudaGetLastError() != cudaSuccess) return LINATTN_ERR_CUDA;
     return LINATTN_OK;
 }

@@ -20,6 +20,95 @@
 
 namespace linattn {
 
+constexpr int kSimtThreads = 256;
+constexpr int kSimtTokens = 32;  // tokens per chunk
+
+// Eq. 6 for kSimtTokens rows held in x_s (fp32, pitch PITCH) -> phi_s (pitch PITCH).
+// Rows >= valid get phi = 0 so that they add nothing to S, z.  8 threads share one row.
+template <int D>
+__device__ __forceinline__ void feature_map_chunk(const float* __restrict__ x_s, const float* __restrict__ W_s,
+                                                  float* __restrict__ phi_s, int valid)
+{
+    constexpr int M = SimtShape<D>::M, P = (D + 4);
+    constexpr int R = M / 8;  // logits per thread
+    const int tid = threadIdx.x;
+    const int tt = tid >> 3, jl = tid & 7;
+    float u[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) u[r] = 0.f;
+    const float* xr = x_s + tt * P;
+#pragma unroll 4
+    for (int c = 0; c < D; ++c) {
+        const float xv = xr[c];
+#pragma unroll
+        for (int r = 0; r < R; ++r) u[r] = fmaf(xv, W_s[c * M + jl + 8 * r], u[r]);
+    }
+    float umax = u[0], umin = u[0];
+#pragma unroll
+    for (int r = 1; r < R; ++r) { umax = fmaxf(umax, u[r]); umin = fminf(umin, u[r]); }
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) {
+        umax = fmaxf(umax, __shfl_xor_sync(0xffffffffu, umax, o));
+        umin = fminf(umin, __shfl_xor_sync(0xffffffffu, umin, o));
+    }
+    float ep[R], en[R], sp = 0.f, sn = 0.f;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        ep[r] = expf(u[r] - umax);   // softmax(+u), max-subtracted
+        en[r] = expf(umin - u[r]);   // softmax(-u): max(-u) = -min(u)
+        sp += ep[r];
+        sn += en[r];
+    }
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) {
+        sp += __shfl_xor_sync(0xffffffffu, sp, o);
+        sn += __shfl_xor_sync(0xffffffffu, sn, o);
+    }
+    const float keep = (tt < valid) ? 1.f : 0.f;
+    const float ip = keep / sp, in = keep / sn;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        phi_s[tt * P + jl + 8 * r] = ep[r] * ip;
+        phi_s[tt * P + M + jl + 8 * r] = en[r] * in;
+    }
+}
+
+// The ReLU kernel function, phi(x) = max(x, 0) element by element, for the chunk; rows >= valid get phi = 0.
+template <int D>
+__device__ __forceinline__ void relu_chunk(const float* __restrict__ x_s, float* __restrict__ phi_s, int valid)
+{
+    constexpr int P = (D + 4);
+    for (int e = threadIdx.x; e < kSimtTokens * D; e += kSimtThreads) {
+        const int r = e / D, c = e % D;
+        phi_s[r * P + c] = (r < valid) ? fmaxf(x_s[r * P + c], 0.f) : 0.f;
+    }
+}
+
+// Load `rows` x D elements starting at src (row-major, contiguous) into dst (fp32, pitch PITCH);
+// rows in [valid, kSimtTokens) are zero-filled.
+template <typename T, int D>
+__device__ __forceinline__ void load_chunk(const T* __restrict__ src, long long row_stride, float* __restrict__ dst, int valid)
+{
+    constexpr int P = (D + 4);
+    for (int e = threadIdx.x; e < kSimtTokens * D; e += kSimtThreads) {
+        const int r = e / D, c = e % D;
+        dst[r * P + c] = (r < valid) ? to_f32(src[(size_t)r * row_stride + c]) : 0.f;
+    }
+}
+
+// state[g][e] = sum_{s=0..splits-1} partial[g][s][e], s ascending.  grid = (ceil(E/256), G), E = D*D + D.
+static __global__ void __launch_bounds__(256)
+combine_blocks(const float* __restrict__ partial, float* __restrict__ state, int splits, int E)
+{
+    const int e = blockIdx.x * 256 + threadIdx.x;
+    if (e >= E) return;
+    const int g = blockIdx.y;
+    const float* p = partial + (size_t)g * splits * E + e;
+    float acc = 0.f;
+    for (int s = 0; s < splits; ++s) acc += p[(size_t)s * E];
+    state[(size_t)g * E + e] = acc;
+}
+
 template <int D> struct BwdShape {
     static constexpr int M = D / 2;
     static constexpr int P = D + 4;    // pitch of token-major tiles and of the state matrix in shared memory
