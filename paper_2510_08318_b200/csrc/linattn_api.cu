@@ -258,22 +258,18 @@ linattn_status launch_backward_simt(linattn_ctx* c, const void* q, const void* k
     const long long G = (long long)B * c->H;
     const int forced = forced_splits(n, c->opt_splits);
     const SimtRuns rk = kside_runs<D>(G, n, forced);
-    const int nchunks = (n + kSimtTokens - 1) / kSimtTokens;
-    long long blocks = (kTargetCtas + G - 1) / G;   // blocks per (b,h) of the two gradient kernels
-    if (blocks > nchunks) blocks = nchunks;
-    if (G * forced > c->partial_slots || G * blocks > c->partial_slots) return LINATTN_ERR_WORKSPACE;
-    constexpr int E = D * D + D, DM = D * (D / 2);
+    const SimtRuns rb = bwd_runs<D>(G, n);
+    if (G * forced > c->partial_slots || rb.P + G - 1 > c->partial_slots) return LINATTN_ERR_WORKSPACE;
+    constexpr int DM = D * (D / 2);
 
     bool& attr_done = c->attr_done[linattn_ctx::kAttrSimtBwd + (sizeof(T) == 2 ? 2 : 0) + (D == 128 ? 1 : 0)];
     if (!attr_done) {
         LA_CUDA(c, (simt_forward_attributes<T, D>()));
-        LA_CUDA(c, cudaFuncSetAttribute(qside_bwd<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bwd_smem<D>()));
-        LA_CUDA(c, cudaFuncSetAttribute(kside_bwd<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bwd_smem<D>()));
+        LA_CUDA(c, (simt_backward_attributes<T, D>()));
         attr_done = true;
     }
     const ActStrides as = act_strides(c, n);
     const double tensor_bytes = (double)G * n * D * sizeof(T);
-    const dim3 grid((unsigned)blocks, (unsigned)G);
     prof_begin(c, st);
     const int relu = c->opt_phi;
     launch_kside_simt<T, D>(rk, (const T*)k, (const T*)v, c->Wk, c->partial, c->H, n, as, relu, st);
@@ -282,32 +278,35 @@ linattn_status launch_backward_simt(linattn_ctx* c, const void* q, const void* k
     launch_combine_state<D>(rk, c->partial, c->state, G, st);
     LA_CUDA(c, cudaGetLastError());
     prof_mark(c, st, "combine_state", 0.0);
-    qside_bwd<T, D><<<grid, kSimtThreads, bwd_smem<D>(), st>>>((const T*)q, (const T*)dout, c->Wq, c->state, (T*)dq,
-                                                              c->bwd_part_state, c->bwd_part_w, c->H, n, as, relu, (const T*)mg.a,
-                                                              mg.lin_scale, mg.dr ? c->bwd_part_dr : nullptr);
+    auto* const q_kernel = rb.small ? qside_bwd<T, D, 1> : qside_bwd<T, D, 4>;
+    auto* const k_kernel = rb.small ? kside_bwd<T, D, 1> : kside_bwd<T, D, 4>;
+    constexpr unsigned threads = 32 * kSimtBwdWarps;
+    q_kernel<<<(unsigned)rb.P, threads, rb.small ? simt_bwd_smem<D, 1, true>() : simt_bwd_smem<D, 4, true>(), st>>>(
+        (const T*)q, (const T*)dout, c->Wq, c->state, (T*)dq, c->bwd_part_state, c->bwd_part_w, c->H, n, rb.Tn, rb.tiles, as, relu,
+        (const T*)mg.a, mg.lin_scale, mg.dr ? c->bwd_part_dr : nullptr);
     LA_CUDA(c, cudaGetLastError());
     prof_mark(c, st, "qside_bwd", 3.0 * tensor_bytes);
     int launches = 5;
-    combine_blocks<<<dim3((E + 255) / 256, (unsigned)G), 256, 0, st>>>(c->bwd_part_state, c->bwd_dstate, (int)blocks, E);
+    launch_combine_state<D>(rb, c->bwd_part_state, c->bwd_dstate, G, st);
     LA_CUDA(c, cudaGetLastError());
-    const dim3 wgrid((DM + 255) / 256, per_head ? (unsigned)c->H : 1u);
+    const dim3 wgrid(DM / 256, per_head ? (unsigned)c->H : 1u);
     if (!relu) {   // the ReLU kernel function has no weights
-        combine_wgrad<<<wgrid, 256, 0, st>>>(c->bwd_part_w, dWq, (int)blocks, (int)G, c->H, DM, per_head);
+        combine_wgrad<<<wgrid, 512, 0, st>>>(c->bwd_part_w, dWq, (int)G, c->H, DM, per_head, rb.Tn, rb.tiles, rb.P);
         LA_CUDA(c, cudaGetLastError());
         ++launches;
     }
     if (mg.dr) {
-        combine_dr<<<1, 32, 0, st>>>(c->bwd_part_dr, (int)(G * blocks), mg.r_in_range, mg.dr);
+        combine_dr<<<1, 32, 0, st>>>(c->bwd_part_dr, (int)rb.P, mg.r_in_range, mg.dr);
         LA_CUDA(c, cudaGetLastError());
         ++launches;
     }
     prof_mark(c, st, "combine_dstate_dWq", 0.0);
-    kside_bwd<T, D><<<grid, kSimtThreads, bwd_smem<D>(), st>>>((const T*)k, (const T*)v, c->Wk, c->bwd_dstate, (T*)dk, (T*)dv,
-                                                              c->bwd_part_w, c->H, n, as, relu);
+    k_kernel<<<(unsigned)rb.P, threads, rb.small ? simt_bwd_smem<D, 1, false>() : simt_bwd_smem<D, 4, false>(), st>>>(
+        (const T*)k, (const T*)v, c->Wk, c->bwd_dstate, (T*)dk, (T*)dv, c->bwd_part_w, c->H, n, rb.Tn, rb.tiles, as, relu);
     LA_CUDA(c, cudaGetLastError());
     prof_mark(c, st, "kside_bwd", 4.0 * tensor_bytes);
     if (!relu) {
-        combine_wgrad<<<wgrid, 256, 0, st>>>(c->bwd_part_w, dWk, (int)blocks, (int)G, c->H, DM, per_head);
+        combine_wgrad<<<wgrid, 512, 0, st>>>(c->bwd_part_w, dWk, (int)G, c->H, DM, per_head, rb.Tn, rb.tiles, rb.P);
         LA_CUDA(c, cudaGetLastError());
         ++launches;
     }

@@ -74,8 +74,9 @@ struct ActStrides {
 __host__ __device__ __forceinline__ long long run_begin(long long p, long long T, long long P) { return p * T / P; }
 
 // acc[i][:] += sum_k a_i[k] * b[k][:]  for this thread's TM rows a_i (a + i * a_step, k contiguous) and NB groups of four
-// columns (b + nb * b_step); accumulator pairs run along the columns.
-template <int K, int TM, int NB>
+// columns (b + nb * b_step); accumulator pairs run along the columns.  SPREAD: row k of b is kept at row
+// (k / M) M + (k % 4) M/4 + (k % M) / 4 with M = K/2 (the gradient kernels' order of W and of the state).
+template <int K, int TM, int NB, bool SPREAD = false>
 __device__ __forceinline__ void rows_times_matrix(const float* __restrict__ a, int a_step, const float* __restrict__ b, int pb,
                                                   int b_step, f32x2 (&acc)[TM][2 * NB])
 {
@@ -84,11 +85,12 @@ __device__ __forceinline__ void rows_times_matrix(const float* __restrict__ a, i
         float4 av[TM];
 #pragma unroll
         for (int i = 0; i < TM; ++i) av[i] = *reinterpret_cast<const float4*>(a + i * a_step + k);
+        const int row0 = (k / (K / 2)) * (K / 2) + (k % (K / 2)) / 4;
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
             ulonglong2 bv[NB];
 #pragma unroll
-            for (int nb = 0; nb < NB; ++nb) bv[nb] = *reinterpret_cast<const ulonglong2*>(b + (k + kk) * pb + nb * b_step);
+            for (int nb = 0; nb < NB; ++nb) bv[nb] = *reinterpret_cast<const ulonglong2*>(b + (SPREAD ? row0 + kk * (K / 8) : k + kk) * pb + nb * b_step);
 #pragma unroll
             for (int i = 0; i < TM; ++i) {
                 const f32x2 x = pack2(part(av[i], kk), part(av[i], kk));
@@ -176,8 +178,8 @@ template <int JG> __device__ __forceinline__ float group_sum(float x)
 // phi of this thread's tokens, TM x 8 values in registers: p[i][j] is feature 4 jg + j, p[i][4 + j] feature M + 4 jg + j of
 // token tg + TG * i (jg = lane % JG).  x: the token group's first row of the tile (warp-private rows); W_s: pitch PW.
 // Hedgehog: Eq. 6 with both softmaxes shifted by their maximum; relu: max(x, 0).  Rows >= valid get phi = 0 (they add
-// nothing to S, z).  1 / sum is applied by multiplication, as one division per row and softmax.
-template <int D, int TG, int TM>
+// nothing to S, z).  1 / sum is applied by multiplication, as one division per row and softmax.  SPREAD: see rows_times_matrix.
+template <int D, int TG, int TM, bool SPREAD = false>
 __device__ __forceinline__ void feature_map_rows(const float* __restrict__ x, const float* __restrict__ W_s, int tg, int jg,
                                                  int valid, int relu, float (&p)[TM][8])
 {
@@ -195,7 +197,7 @@ __device__ __forceinline__ void feature_map_rows(const float* __restrict__ x, co
     }
     f32x2 acc[TM][2];
     zero_acc(acc);
-    rows_times_matrix<D, TM, 1>(x, TG * PX, W_s + 4 * jg, PW, 0, acc);
+    rows_times_matrix<D, TM, 1, SPREAD>(x, TG * PX, W_s + 4 * jg, PW, 0, acc);
 #pragma unroll
     for (int i = 0; i < TM; ++i) {
         float u[4];

@@ -57,3 +57,56 @@ def test_forced_splits(splits):
         ctx.check()
         check(out.cpu().numpy(), oracle.ref_linear(x["q"], x["k"], x["v"], x["Wq"], x["Wk"]), f"splits={splits} n={n}")
         ctx.destroy()
+
+
+# gradients: tiles of 16 / 32 tokens while the large ones (64 / 128) number fewer than 148, then the large form; ragged last
+# tiles, runs that cross pairs
+BWD_SHAPES = [(1, 2, 2), (1, 3, 15), (2, 1, 17), (1, 2, 33), (2, 3, 777), (1, 3, 3201), (2, 2, 5003)]
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("B,H,n", BWD_SHAPES, ids=[f"B{b}H{h}n{n}" for b, h, n in BWD_SHAPES])
+def test_backward_tiles_and_runs(B, H, n, d):
+    """A gradient passes through two more products than the output (dphi, then dx or dW): twice the bound."""
+    x = synth.make_inputs(1, B=B, H=H, n=n, d=d)
+    dout = torch.randn(B, H, n, d, generator=torch.Generator().manual_seed(n))
+    want = oracle.ref_backward(x["q"], x["k"], x["v"], x["Wq"], x["Wk"], dout)
+    ctx = linattn.LinAttn(H, d, max_B=B, max_n=n)
+    ctx.set_feature_map(x["Wq"].cuda(), x["Wk"].cuda())
+    args = [x[t].cuda() for t in ("q", "k", "v")] + [dout.cuda()]
+    got = ctx.backward(*args)
+    ctx.check()
+    for name, g, w in zip(("dq", "dk", "dv", "dWq", "dWk"), got, want):
+        rel, _ = errors(g.cpu().numpy(), w)
+        assert rel <= 2 * TOL, f"{name}: rel-L2 {rel:.2e}"
+    again = ctx.backward(*args)
+    assert all(torch.equal(a, b) for a, b in zip(got, again))
+    ctx.destroy()
+
+
+@pytest.mark.parametrize("d,n", [(128, 3201), (64, 100)])
+def test_shared_weight_gradients_and_other_kernel_function(d, n):
+    """One matrix for eleven heads (every slice of the weight-gradient sum takes whole pairs), and the ReLU kernel function's
+    gradients, token-major, against the oracle."""
+    H = 11
+    x = synth.make_inputs(1, B=1, H=H, n=n, d=d)
+    dout = torch.randn(1, H, n, d, generator=torch.Generator().manual_seed(n))
+    ctx = linattn.LinAttn(H, d, max_B=1, max_n=n)
+    ctx.set_feature_map(x["Wq"][0].contiguous().cuda(), x["Wk"][0].contiguous().cuda())
+    args = [x[t].cuda() for t in ("q", "k", "v")] + [dout.cuda()]
+    got = ctx.backward(*args, per_head=False)
+    ctx.check()
+    want = oracle.ref_backward(x["q"], x["k"], x["v"], x["Wq"][0], x["Wk"][0], dout)
+    for name, g, w in zip(("dq", "dk", "dv", "dWq", "dWk"), got, want):
+        assert errors(g.cpu().numpy(), w)[0] <= 2 * TOL, name
+    ctx.set_option(linattn.OPT_KERNEL_FUNCTION, linattn.PHI_RELU)
+    ctx.set_option(linattn.OPT_LAYOUT, linattn.LAYOUT_BNHD)
+    tm = [a.transpose(1, 2).contiguous().view(1, H, n, d) for a in args]
+    got = ctx.backward(*tm)
+    ctx.check()
+    want = oracle.ref_relu_backward(x["q"], x["k"], x["v"], dout)
+    for name, g, w in zip(("dq", "dk", "dv"), got, want):
+        # a query whose phi meets few keys' divides by a small denominator: the bound on a row grows with 1 / den
+        g = g.view(1, n, H, d).transpose(1, 2)
+        assert errors(g.cpu().numpy(), w)[0] <= 4 * TOL, name
+    ctx.destroy()
