@@ -137,11 +137,13 @@ linattn_status linattn_forward_mixed(linattn_ctx* ctx, const void* q, const void
  *   dWq, dWk      : device, fp32, 16-byte aligned, written in full: [H][d][d/2] when per_head != 0 (each head's
  *                   gradient summed over the batch), [d][d/2] when per_head == 0 (one shared matrix: summed over
  *                   batch and heads).  The weights differentiated are the ones given to set_feature_map.
- * Two sets of kernels, chosen like the forward's (LINATTN_OPT_PATH): for bf16 activations with d = 128 and bf16
- * feature-map weights the products run on the tensor cores (bf16 operands, fp32 accumulation; S and dS enter as
- * bf16 hi + lo pairs and dO itself, exact in bf16, is the operand where dO / den is needed, so that gradients stay
- * accurate when V has a large mean; relative L2 error about 3e-3 per gradient); everything else, or path 1, runs in
- * fp32 on the CUDA cores (the stored q, k, v, dout are then the only rounded quantities).  dq, dk, dv are
+ * Three sets of kernels.  bf16 activations with d = 128 and bf16 feature-map weights: the products run on the tensor cores
+ * with bf16 operands and fp32 accumulation (S and dS enter as bf16 hi + lo pairs and dO itself, exact in bf16, is the
+ * operand where dO / den is needed, so that gradients stay accurate when V has a large mean; relative L2 error about 3e-3
+ * per gradient).  bf16 activations with d = 64 or fp32 weights: at fp32 accuracy (the stored q, k, v, dout are then the
+ * only rounded quantities), on the tensor cores with every computed operand as a sum of three bf16 parts when there is
+ * enough work, else on the CUDA cores.  fp32 activations, the ReLU kernel function, or LINATTN_OPT_PATH = 1: in fp32 on the
+ * CUDA cores.  LINATTN_OPT_PATH = 2 asks for the first set and is an error where it does not apply.  dq, dk, dv are
  * rounded once to `dtype`.  All sums have a fixed order: the same inputs give bit-identical gradients.  The first
  * call allocates the backward workspace (it synchronises the device once); later calls allocate nothing.  After
  * the call the context holds the S, z of these k, v (linattn_read_state returns them).

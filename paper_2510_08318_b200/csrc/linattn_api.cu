@@ -17,6 +17,7 @@
 #include "simt_backward.cuh"
 #include "sm100_kernels.cuh"
 #include "sm100_backward.cuh"
+#include "sm100_split_backward.cuh"
 #include "tensor_map.hpp"
 
 using namespace linattn;
@@ -62,6 +63,8 @@ struct linattn_ctx {
     __nv_bfloat16* Wkt = nullptr;
     __nv_bfloat16* Wqt_lo = nullptr;   // what the bf16 rounding of fp32 weights leaves, rounded to bf16 again: W = hi + lo
     __nv_bfloat16* Wkt_lo = nullptr;
+    __nv_bfloat16* Wqt_lo2 = nullptr;  // and what that leaves: W = hi + lo + lo2 to 2^-26 (the gradients at fp32 accuracy)
+    __nv_bfloat16* Wkt_lo2 = nullptr;
     bool map_is_bf16 = false;   // the caller supplied bf16 weights: the images above are exact and the lo parts unused
     __nv_bfloat16* s_img = nullptr;  // [max_B*H][128*128] bf16 image of S for the query-side TMA
     __nv_bfloat16* z_img = nullptr;  // [max_B*H][2048] bf16 operand image of z (hi, lo)
@@ -76,12 +79,13 @@ struct linattn_ctx {
     float* state = nullptr;     // [max_B*H][d*d + d]
     unsigned int* err_word = nullptr;
     // workspace of the backward pass, allocated by the first linattn_backward
-    float* bwd_part_state = nullptr;  // [partial_slots][d*d + d]  per-block sums of dS, dz
-    float* bwd_part_w = nullptr;      // [partial_slots][d*d/2]    per-block sums of dW
+    float* bwd_part_state = nullptr;  // [partial_slots][128*128 + 128]  per-block sums of dS, dz
+    float* bwd_part_w = nullptr;      // [partial_slots][128*64]         per-block sums of dW
     float* bwd_part_w2 = nullptr;     // the same for dW_k on the tensor-core path (both weight gradients are summed by one launch at the end)
     float* bwd_dstate = nullptr;      // [max_B*H][d*d + d]        dS, dz
     float* bwd_part_dr = nullptr;     // [partial_slots]           per-block sums of dout . (a - o), the terms of Eq. 8's dL/dr
-    __nv_bfloat16* bwd_img[3] = {nullptr, nullptr, nullptr};   // tensor-core backward: lo image of S, hi and lo images of dS
+    __nv_bfloat16* bwd_img[3] = {nullptr, nullptr, nullptr};   // tensor-core backward: lo image of S, hi and lo images of dS; at fp32 accuracy: the three parts of S, then of dS
+    float* bwd_vec = nullptr;         // [units][128]              z, then dz, of each 128-feature unit (gradients at fp32 accuracy)
     bool bwd_ready = false;           // every allocation above succeeded
     // host-call staging and its pipeline: copies in, compute and copies out run on three streams, one (b,h) at a time
     void* stage[4] = {nullptr, nullptr, nullptr, nullptr};
@@ -122,7 +126,7 @@ struct linattn_ctx {
     // bookkeeping
     // shared-memory limit raised on this context's device, per kernel family (function attributes are per device)
     enum AttrSlot { kAttrSimtFwd = 0 /* +0..3: (storage type, head dim) */, kAttrSimtBwd = 4 /* +0..3 */, kAttrTcFwd = 8,
-                    kAttrTcBwd = 9, kAttrSlots = 10 };
+                    kAttrTcBwd = 9, kAttrSplitBwd = 10, kAttrSlots = 11 };
     bool attr_done[kAttrSlots] = {};
     int last_launches = 0;
     int last_B = 0;
@@ -583,6 +587,133 @@ linattn_status launch_backward_tc(linattn_ctx* c, const void* q, const void* k, 
     return LINATTN_OK;
 }
 
+// Whether bf16 activations whose gradients need fp32 accuracy (d = 64, or fp32 weights) go to the tensor-core kernels or to the
+// CUDA-core ones.  A tile costs the former about 14 us in each gradient kernel whatever the number of tiles, so few tiles
+// leave them behind the small tiles of the latter (d = 128, measured per backward: 12 tiles 89 / 78 us, 27 tiles 89 / 117 us,
+// 66 tiles 89 / 158 us).  Their error against 64 bits does not depend on n (dW 4.1e-7 to 4.6e-7 at d = 64, 5.8e-7 to 6.2e-7 at
+// d = 128), that of sums kept in fp32 registers grows with it and is the smaller one for short sequences of 64-feature heads
+// (3.3e-7 at n = 200, 4.9e-7 at 1100, 1.1e-6 at 14040): those stay where they were.
+bool split_backward_pays(const linattn_ctx* c, long long heads, int n)
+{
+    const long long units = c->d == 64 ? (heads + 1) / 2 : heads;
+    const long long tiles = units * (((long long)n + tc::kTile - 1) / tc::kTile);
+    return c->d == 64 ? (tiles >= c->num_sms && n >= 1024) : tiles >= 24;
+}
+
+// Gradients on the tensor cores at fp32 accuracy (bf16 activations; d = 64, or fp32 feature-map weights): S, z, then the query
+// side (dq; dS, dz, dW_q records), the combines, and the key side (dk, dv; dW_k records).
+linattn_status launch_backward_split(linattn_ctx* c, const void* q, const void* k, const void* v, const void* dout, void* dq, void* dk, void* dv,
+                                     float* dWq, float* dWk, int per_head, int B, int n, cudaStream_t st, const MixGrad& mg)
+{
+    using namespace linattn::tc;
+    const int pair = c->d == 64 ? 1 : 0;
+    const long long heads = (long long)B * c->H, units = pair ? (heads + 1) / 2 : heads;
+    const long long Tn = ((long long)n + kTile - 1) / kTile, T = units * Tn;
+    const long long P = c->num_sms < T ? c->num_sms : T;
+    if (P + units > c->partial_slots_tc) return LINATTN_ERR_WORKSPACE;
+    const ActStrides as = act_strides(c, n);
+    const int layout = c->opt_layout;
+    auto act_map = [&](CUtensorMap* m, const void* base) {
+        if (layout == 0) return make_tmap_bf16_3d(m, base, (uint64_t)c->d, (uint64_t)n, (uint64_t)heads, kTile);
+        return make_tmap_bf16_act(m, base, (uint64_t)c->d, (uint64_t)n, (uint64_t)c->H, (uint64_t)B, (uint64_t)as.token * 2,
+                                  (uint64_t)as.head * 2, (uint64_t)as.batch * 2, kTile);
+    };
+    auto w_map = [&](CUtensorMap* m, const void* base) { return make_tmap_bf16_3d(m, base, kD, kM, (uint64_t)c->H, kM); };
+    CUtensorMap tmQ, tmG, tmDQ, tmK, tmV, tmDK, tmDV, tmWq[3], tmWk[3], tmImg[3];
+    bool ok = act_map(&tmQ, q) && act_map(&tmG, dout) && act_map(&tmDQ, dq) && act_map(&tmK, k) && act_map(&tmV, v) && act_map(&tmDK, dk) &&
+              act_map(&tmDV, dv) && w_map(&tmWq[0], c->Wqt) && w_map(&tmWq[1], c->Wqt_lo) && w_map(&tmWq[2], c->Wqt_lo2) &&
+              w_map(&tmWk[0], c->Wkt) && w_map(&tmWk[1], c->Wkt_lo) && w_map(&tmWk[2], c->Wkt_lo2);
+    for (int i = 0; i < 3; ++i) ok = ok && make_tmap_bf16_3d(&tmImg[i], c->bwd_img[i], kD, kD, (uint64_t)units, kTile);
+    if (!ok) {
+        snprintf(c->err_text, sizeof(c->err_text), "cuTensorMapEncodeTiled failed");
+        return LINATTN_ERR_CUDA;
+    }
+    // [layout][pair]([Eq. 8 terms])
+    static const void* const k_s[2][2] = {{(const void*)kside_split_tc<0, 0>, (const void*)kside_split_tc<0, 1>},
+                                          {(const void*)kside_split_tc<1, 0>, (const void*)kside_split_tc<1, 1>}};
+    static const void* const k_q[2][2][2] = {{{(const void*)qside_bwd_split_tc<0, 0, 0>, (const void*)qside_bwd_split_tc<0, 0, 1>},
+                                              {(const void*)qside_bwd_split_tc<0, 1, 0>, (const void*)qside_bwd_split_tc<0, 1, 1>}},
+                                             {{(const void*)qside_bwd_split_tc<1, 0, 0>, (const void*)qside_bwd_split_tc<1, 0, 1>},
+                                              {(const void*)qside_bwd_split_tc<1, 1, 0>, (const void*)qside_bwd_split_tc<1, 1, 1>}}};
+    static const void* const k_k[2][2] = {{(const void*)kside_bwd_split_tc<0, 0>, (const void*)kside_bwd_split_tc<0, 1>},
+                                          {(const void*)kside_bwd_split_tc<1, 0>, (const void*)kside_bwd_split_tc<1, 1>}};
+    bool& attr_done = c->attr_done[linattn_ctx::kAttrSplitBwd];
+    if (!attr_done) {
+        const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+        for (int i = 0; i < 2; ++i) {
+            LA_CUDA(c, cudaFuncSetAttribute(k_s[i][pair], at, (int)kSpSmemState));
+            LA_CUDA(c, cudaFuncSetAttribute(k_k[i][pair], at, (int)kSpSmem));
+            for (int j = 0; j < 2; ++j) LA_CUDA(c, cudaFuncSetAttribute(k_q[i][pair][j], at, (int)kSpSmem));
+        }
+        attr_done = true;
+    }
+    SpArgs a{};
+    a.rec = c->partial;
+    a.rec_w = c->bwd_part_w;
+    a.vec = c->bwd_vec;
+    a.err = c->err_word;
+    a.mix_a = (const __nv_bfloat16*)mg.a;
+    a.part_dr = c->bwd_part_dr;
+    a.lin_scale = mg.lin_scale;
+    a.str_token = as.token;
+    a.str_head = as.head;
+    a.str_batch = as.batch;
+    a.n = n;
+    a.H = c->H;
+    a.heads = (int)heads;
+    a.tiles_per_unit = (int)Tn;
+    a.total_tiles = T;
+    a.w_parts = c->map_is_bf16 ? 1 : 3;
+    a.wait_limit_us = (uint32_t)c->opt_wait_limit_us;
+    const double tensor_bytes = (double)heads * n * c->d * 2;
+    const dim3 grid((unsigned)P), block(kSpThreads), cgrid((kE + 255) / 256, (unsigned)units);
+    const dim3 wgrid((unsigned)(c->d * c->d / 2 + 255) / 256, per_head ? (unsigned)c->H : 1u);
+    auto combine = [&](const float* rec, float* state) {
+        if (pair) combine_split<1><<<cgrid, 256, 0, st>>>(rec, c->bwd_img[0], c->bwd_img[1], c->bwd_img[2], c->bwd_vec, state, (int)heads, (int)Tn, T, P);
+        else combine_split<0><<<cgrid, 256, 0, st>>>(rec, c->bwd_img[0], c->bwd_img[1], c->bwd_img[2], c->bwd_vec, state, (int)heads, (int)Tn, T, P);
+        return cudaGetLastError();
+    };
+    auto combine_w = [&](float* dW) {
+        if (pair) combine_wgrad_split<1><<<wgrid, 256, 0, st>>>(c->bwd_part_w, dW, (int)heads, c->H, per_head, (int)Tn, T, P);
+        else combine_wgrad_split<0><<<wgrid, 256, 0, st>>>(c->bwd_part_w, dW, (int)heads, c->H, per_head, (int)Tn, T, P);
+        return cudaGetLastError();
+    };
+    int launches = 7;
+    prof_begin(c, st);
+    {
+        void* p[] = {&tmK, &tmV, &tmWk[0], &tmWk[1], &tmWk[2], &a};
+        LA_CUDA(c, cudaLaunchKernel(k_s[layout][pair], grid, block, p, kSpSmemState, st));
+    }
+    prof_mark(c, st, "kside_split_tc", 2.0 * tensor_bytes);
+    LA_CUDA(c, combine(c->partial, c->state));
+    prof_mark(c, st, "combine_state", 0.0);
+    a.rec = c->bwd_part_state;
+    a.test_unmet = c->opt_unmet == 2 ? 1 : 0;
+    {
+        void* p[] = {&tmQ, &tmG, &tmDQ, &tmWq[0], &tmWq[1], &tmWq[2], &tmImg[0], &tmImg[1], &tmImg[2], &a};
+        LA_CUDA(c, cudaLaunchKernel(k_q[layout][pair][mg.dr ? 1 : 0], grid, block, p, kSpSmem, st));
+    }
+    prof_mark(c, st, "qside_bwd_split_tc", (mg.dr ? 4.0 : 3.0) * tensor_bytes);
+    if (mg.dr) {
+        combine_dr<<<1, 32, 0, st>>>(c->bwd_part_dr, (int)P, mg.r_in_range, mg.dr);
+        LA_CUDA(c, cudaGetLastError());
+        ++launches;
+    }
+    LA_CUDA(c, combine(c->bwd_part_state, nullptr));
+    LA_CUDA(c, combine_w(dWq));
+    prof_mark(c, st, "combine_dstate_dWq", 0.0);
+    a.test_unmet = c->opt_unmet == 3 ? 1 : 0;
+    {
+        void* p[] = {&tmK, &tmV, &tmDK, &tmDV, &tmWk[0], &tmWk[1], &tmWk[2], &tmImg[0], &tmImg[1], &tmImg[2], &a};
+        LA_CUDA(c, cudaLaunchKernel(k_k[layout][pair], grid, block, p, kSpSmem, st));
+    }
+    prof_mark(c, st, "kside_bwd_split_tc", 4.0 * tensor_bytes);
+    LA_CUDA(c, combine_w(dWk));
+    prof_mark(c, st, "combine_dWk", 0.0);
+    c->last_launches = launches;
+    return LINATTN_OK;
+}
+
 bool misaligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) != 0; }
 
 bool overlaps(const void* a, const void* b, size_t bytes)
@@ -662,10 +793,15 @@ linattn_status linattn_create(linattn_ctx** out_ctx, int device, int H, int d, l
     if (e == cudaSuccess) {
         // weight images W^T [H][64][128] bf16 (d = 64: of each pair of consecutive heads), bf16 image of S and operand image of z per unit
         const size_t wt = sizeof(__nv_bfloat16) * (size_t)H * linattn::tc::kM * linattn::tc::kD;
-        e = cudaMalloc(&c->Wqt, wt);
-        if (e == cudaSuccess) e = cudaMalloc(&c->Wkt, wt);
-        if (e == cudaSuccess) e = cudaMalloc(&c->Wqt_lo, wt);
-        if (e == cudaSuccess) e = cudaMalloc(&c->Wkt_lo, wt);
+        e = cudaMalloc(&c->Wqt, 6 * wt);   // [part][query, key]: one allocation
+        if (e == cudaSuccess) {
+            const size_t plane = wt / sizeof(__nv_bfloat16);
+            c->Wkt = c->Wqt + plane;
+            c->Wqt_lo = c->Wqt + 2 * plane;
+            c->Wkt_lo = c->Wqt + 3 * plane;
+            c->Wqt_lo2 = c->Wqt + 4 * plane;
+            c->Wkt_lo2 = c->Wqt + 5 * plane;
+        }
         if (e == cudaSuccess) e = cudaMalloc(&c->s_img, sizeof(__nv_bfloat16) * (size_t)G * linattn::tc::kD * linattn::tc::kD);
         if (e == cudaSuccess) e = cudaMalloc(&c->z_img, (size_t)G * linattn::tc::kZBlkBytes);
         if (e == cudaSuccess) e = cudaMemset(c->z_img, 0, (size_t)G * linattn::tc::kZBlkBytes);
@@ -702,9 +838,7 @@ linattn_status linattn_destroy(linattn_ctx* c)
     cudaFree(c->err_word);
     cudaFree(c->sync_words);
     cudaFree(c->Wqt);
-    cudaFree(c->Wkt);
-    cudaFree(c->Wqt_lo);
-    cudaFree(c->Wkt_lo);
+    cudaFree(c->bwd_vec);
     cudaFree(c->s_img);
     cudaFree(c->z_img);
     cudaFree(c->bwd_part_state);
@@ -737,35 +871,18 @@ linattn_status linattn_set_feature_map(linattn_ctx* c, const void* Wq, const voi
     const int DM = c->d * (c->d / 2);
     const size_t total = (size_t)c->H * DM;
     const unsigned blocks = (unsigned)((total + 255) / 256);
-    if (wdtype == LINATTN_F32) {
-        convert_weights<float><<<blocks, 256, 0, st>>>((const float*)Wq, c->Wq, c->H, DM, per_head ? 1 : 0);
-        convert_weights<float><<<blocks, 256, 0, st>>>((const float*)Wk, c->Wk, c->H, DM, per_head ? 1 : 0);
-    } else {
-        convert_weights<__nv_bfloat16><<<blocks, 256, 0, st>>>((const __nv_bfloat16*)Wq, c->Wq, c->H, DM, per_head ? 1 : 0);
-        convert_weights<__nv_bfloat16><<<blocks, 256, 0, st>>>((const __nv_bfloat16*)Wk, c->Wk, c->H, DM, per_head ? 1 : 0);
-    }
-    {
-        // images for the tensor-core kernels: W^T [H][64][128] bf16 (d = 64: of each pair of consecutive heads); fp32 weights
-        // are kept as a bf16 hi + lo pair
-        const unsigned tb = (unsigned)(((size_t)c->H * tc::kM * tc::kD + 255) / 256);
-        const int ph = per_head ? 1 : 0;
-        auto images = [&](auto src_q, auto src_k) {
-            using T = std::remove_cv_t<std::remove_pointer_t<decltype(src_q)>>;
-            for (int lo = 0; lo < (wdtype == LINATTN_F32 ? 2 : 1); ++lo) {
-                __nv_bfloat16* dq = lo ? c->Wqt_lo : c->Wqt;
-                __nv_bfloat16* dk = lo ? c->Wkt_lo : c->Wkt;
-                if (c->d == 64) {
-                    tc::pair_weights_bf16<T><<<tb, 256, 0, st>>>(src_q, dq, c->H, ph, lo);
-                    tc::pair_weights_bf16<T><<<tb, 256, 0, st>>>(src_k, dk, c->H, ph, lo);
-                } else {
-                    tc::transpose_weights_bf16<T><<<tb, 256, 0, st>>>(src_q, dq, c->H, ph, lo);
-                    tc::transpose_weights_bf16<T><<<tb, 256, 0, st>>>(src_k, dk, c->H, ph, lo);
-                }
-            }
-        };
-        if (wdtype == LINATTN_F32) images((const float*)Wq, (const float*)Wk);
-        else images((const __nv_bfloat16*)Wq, (const __nv_bfloat16*)Wk);
-    }
+    const unsigned tb = (unsigned)(((size_t)c->H * tc::kM * tc::kD + 255) / 256);
+    const int ph = per_head ? 1 : 0, parts = wdtype == LINATTN_F32 ? 3 : 1;
+    // fp32 copies for the CUDA-core kernels, bf16 images for the tensor-core ones (d = 64: of each pair of consecutive heads);
+    // weights given in fp32 are kept as three bf16 parts (the forward reads the first two)
+    auto set = [&](auto src_q, auto src_k) {
+        using T = std::remove_cv_t<std::remove_pointer_t<decltype(src_q)>>;
+        convert_weights<T><<<dim3(blocks, 2), 256, 0, st>>>(src_q, src_k, c->Wq, c->Wk, c->H, DM, ph);
+        if (c->d == 64) tc::weight_images<T, 1><<<dim3(tb, 2), 256, 0, st>>>(src_q, src_k, c->Wqt, c->H, ph, parts);
+        else tc::weight_images<T, 0><<<dim3(tb, 2), 256, 0, st>>>(src_q, src_k, c->Wqt, c->H, ph, parts);
+    };
+    if (wdtype == LINATTN_F32) set((const float*)Wq, (const float*)Wk);
+    else set((const __nv_bfloat16*)Wq, (const __nv_bfloat16*)Wk);
     LA_CUDA(c, cudaGetLastError());
     c->map_is_bf16 = (wdtype == LINATTN_BF16);
     c->have_map = true;
@@ -874,15 +991,16 @@ static linattn_status backward_impl(linattn_ctx* c, const void* q, const void* k
     cudaStream_t st = (cudaStream_t)stream;
     if (!c->bwd_ready) {
         // all or nothing: a failed allocation releases what the earlier ones got, so that the next call starts over
-        const size_t E = (size_t)d * d + d, G = (size_t)(c->max_B * c->H);
-        cudaError_t e = cudaMalloc(&c->bwd_part_state, sizeof(float) * E * (size_t)c->partial_slots);
-        if (e == cudaSuccess) e = cudaMalloc(&c->bwd_part_w, sizeof(float) * (size_t)d * (d / 2) * (size_t)c->partial_slots);
-        if (e == cudaSuccess && d == 128) e = cudaMalloc(&c->bwd_part_w2, sizeof(float) * (size_t)d * (d / 2) * (size_t)c->partial_slots);
+        // the tensor-core kernels' records are those of a 128-feature unit (one head, or a pair of heads of 64), for either d
+        const size_t E = (size_t)d * d + d, G = (size_t)(c->max_B * c->H), units = d == 64 ? (G + 1) / 2 : G;
+        cudaError_t e = cudaMalloc(&c->bwd_part_state, sizeof(float) * (size_t)tc::kE * (size_t)c->partial_slots);
+        if (e == cudaSuccess) e = cudaMalloc(&c->bwd_part_w, sizeof(float) * (size_t)tc::kWRec * (size_t)c->partial_slots);
+        if (e == cudaSuccess) e = cudaMalloc(&c->bwd_part_w2, sizeof(float) * (size_t)tc::kWRec * (size_t)c->partial_slots);
         if (e == cudaSuccess) e = cudaMalloc(&c->bwd_dstate, sizeof(float) * E * G);
         if (e == cudaSuccess) e = cudaMalloc(&c->bwd_part_dr, sizeof(float) * (size_t)c->partial_slots);
-        if (d == 128)
-            for (__nv_bfloat16*& p : c->bwd_img)
-                if (e == cudaSuccess) e = cudaMalloc(&p, sizeof(__nv_bfloat16) * (size_t)d * d * G);
+        if (e == cudaSuccess) e = cudaMalloc(&c->bwd_vec, sizeof(float) * (size_t)tc::kD * units);
+        for (__nv_bfloat16*& p : c->bwd_img)
+            if (e == cudaSuccess) e = cudaMalloc(&p, sizeof(__nv_bfloat16) * (size_t)tc::kD * tc::kD * units);
         if (e != cudaSuccess) {
             cudaGetLastError();
             cudaFree(c->bwd_part_state);
@@ -890,7 +1008,8 @@ static linattn_status backward_impl(linattn_ctx* c, const void* q, const void* k
             cudaFree(c->bwd_part_w2);
             cudaFree(c->bwd_dstate);
             cudaFree(c->bwd_part_dr);
-            c->bwd_part_state = c->bwd_part_w = c->bwd_part_w2 = c->bwd_dstate = c->bwd_part_dr = nullptr;
+            cudaFree(c->bwd_vec);
+            c->bwd_part_state = c->bwd_part_w = c->bwd_part_w2 = c->bwd_dstate = c->bwd_part_dr = c->bwd_vec = nullptr;
             for (__nv_bfloat16*& p : c->bwd_img) {
                 cudaFree(p);
                 p = nullptr;
@@ -909,13 +1028,18 @@ static linattn_status backward_impl(linattn_ctx* c, const void* q, const void* k
         else scale_copy<float><<<blocks, 256, 0, st>>>((const float*)dout, (float*)d_a, count, 1.f - mg.lin_scale);
         LA_CUDA(c, cudaGetLastError());
     }
-    // tensor-core kernels: Eq. 6 with bf16 weights, bf16 activations, d = 128; everything else on the CUDA cores
+    // bf16 activations with Eq. 6 run on the tensor cores: d = 128 with bf16 weights on the kernels with bf16 operands, d = 64
+    // and fp32 weights on those that keep fp32 accuracy (if there is enough work); everything else on the CUDA cores
     const bool tc_ok = (dtype == LINATTN_BF16 && d == 128 && c->map_is_bf16 && !relu);
     if (c->opt_path == 2 && !tc_ok) return LINATTN_ERR_UNSUPPORTED;
     linattn_status res;
     if (tc_ok && c->opt_path != 1) {
         c->state_transposed = true;
         res = launch_backward_tc(c, q, k, v, dout, dq, dk, dv, dWq, dWk, ph, B, n, st, mg);
+    } else if (dtype == LINATTN_BF16 && !relu && c->opt_path != 1 && split_backward_pays(c, (long long)B * H, n)) {
+        c->state_transposed = false;
+        c->state_key.valid = false;
+        res = launch_backward_split(c, q, k, v, dout, dq, dk, dv, dWq, dWk, ph, B, n, st, mg);
     } else {
         c->state_transposed = false;
         c->state_key.valid = false;

@@ -572,14 +572,15 @@ void launch_qside_simt(const SimtRuns& r, const T* q, const float* Wq, const flo
         qside_simt<T, D, kSimtQWarps, 4><<<(unsigned)r.P, 32 * kSimtQWarps, qside_simt_smem<D, kSimtQWarps, 4>(), stream>>>(q, Wq, state, out, H, n, r.Tn, r.tiles, mix, mix_r, st, relu);
 }
 
-// Feature-map weights: any supported storage type -> fp32 [H][D][M]; src is [H][D][M] or, when
-// per_head == 0, a single [D][M] replicated to every head.
+// Feature-map weights: any supported storage type -> fp32 [H][D][M]; src is [H][D][M] or, when per_head == 0, a single
+// [D][M] replicated to every head.  blockIdx.y = 0: W_q, 1: W_k.
 template <typename T>
-__global__ void convert_weights(const T* __restrict__ src, float* __restrict__ dst, int H, int DM, int per_head)
+__global__ void convert_weights(const T* __restrict__ src_q, const T* __restrict__ src_k, float* __restrict__ dst_q, float* __restrict__ dst_k, int H,
+                                int DM, int per_head)
 {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (size_t)H * DM) return;
-    dst[i] = to_f32(src[per_head ? i : i % DM]);
+    (blockIdx.y ? dst_k : dst_q)[i] = to_f32((blockIdx.y ? src_k : src_q)[per_head ? i : i % DM]);
 }
 
 }  // namespace linattn

@@ -1336,42 +1336,34 @@ linattn_fused_tc(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     LA_TRACE_NS(0, 61, 3);
 }
 
-// W [H][128 d][64 j] (any supported type) -> W^T bf16 [H][64 j][128 d]; per_head == 0 replicates one matrix.
-// bf16 hi part of w, or (lo != 0) the bf16 rounding of what the hi part leaves: w = hi + lo to 2^-17 relative.
-__device__ __forceinline__ __nv_bfloat16 bf16_part(float w, int lo)
+// The weight images of the tensor-core kernels, [H][64 j][128 d] bf16, in up to three parts: part 0 is the bf16 rounding of w,
+// part 1 that of what part 0 leaves (w = 0 + 1 to 2^-17 relative), part 2 that of what both leave (2^-26).
+//   d = 128 (kPair = 0): W^T of each head.
+//   d = 64 (kPair = 1): of a PAIR of heads, as the logits MMA of the d = 128 kernels wants it: plane h0 for the pair (h0, h1 =
+//   (h0 + 1) mod H): rows 0..31 hold W_{h0}^T (32 x 64) in columns 0..63 and zeros beside it, rows 32..63 zeros and W_{h1}^T in
+//   columns 64..127, so that [x_{h0}, x_{h1}] (128 features) times its transpose gives [u_{h0} (32 logits), u_{h1} (32 logits)].
+// src: W [H][d][d/2] (any supported type), or one matrix for every head (per_head == 0).  dst: [part][query, key][H][64][128];
+// blockIdx.y = 0: W_q, 1: W_k.
+template <typename T, int kPair>
+static __global__ void __launch_bounds__(256)
+weight_images(const T* __restrict__ Wq, const T* __restrict__ Wk, __nv_bfloat16* __restrict__ dst, int H, int per_head, int parts)
 {
-    const __nv_bfloat16 hi = __float2bfloat16_rn(w);
-    return lo ? __float2bfloat16_rn(w - __bfloat162float(hi)) : hi;
-}
-template <typename T>
-static __global__ void transpose_weights_bf16(const T* __restrict__ src, __nv_bfloat16* __restrict__ dst, int H, int per_head, int lo)
-{
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (size_t)H * kM * kD) return;
+    const size_t plane = (size_t)H * kM * kD, i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= plane) return;
+    const T* src = blockIdx.y ? Wk : Wq;
     const int h = (int)(i / (kM * kD)), rem = (int)(i % (kM * kD)), j = rem / kD, dd = rem % kD;
-    const size_t s = (size_t)(per_head ? h : 0) * kD * kM + (size_t)dd * kM + j;
-    dst[i] = bf16_part((float)src[s], lo);
-}
-
-// Head dimension 64: the weight image of a PAIR of heads, as the logits MMA of the d = 128 kernels wants it.
-// dst [H][64 j'][128 d'] bf16, plane h0 for the pair (h0, h1 = (h0 + 1) mod H):
-//   rows  0..31: W_{h0}^T (32 x 64) in columns 0..63,   zeros in columns 64..127
-//   rows 32..63: zeros in columns 0..63,                W_{h1}^T in columns 64..127
-// so that [x_{h0}, x_{h1}] (128 features) times its transpose gives [u_{h0} (32 logits), u_{h1} (32 logits)].
-// src: W [H][64 d][32 j] (any supported type); per_head == 0: one matrix for every head.
-template <typename T>
-static __global__ void pair_weights_bf16(const T* __restrict__ src, __nv_bfloat16* __restrict__ dst, int H, int per_head, int lo)
-{
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (size_t)H * kM * kD) return;
-    const int h0 = (int)(i / (kM * kD)), rem = (int)(i % (kM * kD)), jp = rem / kD, dp = rem % kD;
-    const int blk = jp >> 5;   // which head of the pair this row of logits belongs to
-    float v = 0.f;
-    if ((dp >> 6) == blk) {
-        const int h = per_head ? (h0 + blk) % H : 0;
-        v = (float)src[(size_t)h * 64 * 32 + (size_t)(dp & 63) * 32 + (jp & 31)];
+    float w = 0.f;
+    if (kPair) {
+        const int blk = j >> 5;   // which head of the pair this row of logits belongs to
+        if ((dd >> 6) == blk) w = (float)src[(size_t)(per_head ? (h + blk) % H : 0) * 64 * 32 + (size_t)(dd & 63) * 32 + (j & 31)];
+    } else {
+        w = (float)src[(size_t)(per_head ? h : 0) * kD * kM + (size_t)dd * kM + j];
     }
-    dst[i] = bf16_part(v, lo);
+    for (int p = 0; p < parts; ++p) {
+        const __nv_bfloat16 b = __float2bfloat16_rn(w);
+        dst[(size_t)(2 * p + blockIdx.y) * plane + i] = b;
+        w -= __bfloat162float(b);
+    }
 }
 
 }  // namespace tc
