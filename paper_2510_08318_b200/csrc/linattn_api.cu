@@ -231,14 +231,11 @@ linattn_status launch_simt(linattn_ctx* c, const void* q, const void* k, const v
     }
     const double side_bytes = 2.0 * (double)G * n * D * sizeof(T);  // K+V read, or Q read + O written
     prof_begin(c, st);
-    launch_kside_simt<T, D>(rk, (const T*)k, (const T*)v, Wk, c->partial, Hv, n, act_strides(c, n), c->opt_phi, st);
-    LA_CUDA(c, cudaGetLastError());
+    LA_CUDA(c, (launch_kside_simt<T, D>(rk, (const T*)k, (const T*)v, Wk, c->partial, Hv, n, act_strides(c, n), c->opt_phi, st)));
     prof_mark(c, st, "kside_simt", side_bytes);
-    launch_combine_state<D>(rk, c->partial, state, G, st);
-    LA_CUDA(c, cudaGetLastError());
+    LA_CUDA(c, (launch_combine_state<D>(rk, c->partial, state, G, st)));
     prof_mark(c, st, "combine_state", 0.0);
-    launch_qside_simt<T, D>(rq, (const T*)q, Wq, state, (T*)out, Hv, n, (const T*)mix, mix_r, act_strides(c, n), c->opt_phi, st);
-    LA_CUDA(c, cudaGetLastError());
+    LA_CUDA(c, (launch_qside_simt<T, D>(rq, (const T*)q, Wq, state, (T*)out, Hv, n, (const T*)mix, mix_r, act_strides(c, n), c->opt_phi, st)));
     prof_mark(c, st, "qside_simt", side_bytes);
     c->last_launches = 3;
     return LINATTN_OK;
@@ -276,42 +273,31 @@ linattn_status launch_backward_simt(linattn_ctx* c, const void* q, const void* k
     const double tensor_bytes = (double)G * n * D * sizeof(T);
     prof_begin(c, st);
     const int relu = c->opt_phi;
-    launch_kside_simt<T, D>(rk, (const T*)k, (const T*)v, c->Wk, c->partial, c->H, n, as, relu, st);
-    LA_CUDA(c, cudaGetLastError());
+    LA_CUDA(c, (launch_kside_simt<T, D>(rk, (const T*)k, (const T*)v, c->Wk, c->partial, c->H, n, as, relu, st)));
     prof_mark(c, st, "kside_simt", 2.0 * tensor_bytes);
-    launch_combine_state<D>(rk, c->partial, c->state, G, st);
-    LA_CUDA(c, cudaGetLastError());
+    LA_CUDA(c, (launch_combine_state<D>(rk, c->partial, c->state, G, st)));
     prof_mark(c, st, "combine_state", 0.0);
     auto* const q_kernel = rb.small ? qside_bwd<T, D, 1> : qside_bwd<T, D, 4>;
     auto* const k_kernel = rb.small ? kside_bwd<T, D, 1> : kside_bwd<T, D, 4>;
     constexpr unsigned threads = 32 * kSimtBwdWarps;
-    q_kernel<<<(unsigned)rb.P, threads, rb.small ? simt_bwd_smem<D, 1, true>() : simt_bwd_smem<D, 4, true>(), st>>>(
-        (const T*)q, (const T*)dout, c->Wq, c->state, (T*)dq, c->bwd_part_state, c->bwd_part_w, c->H, n, rb.Tn, rb.tiles, as, relu,
-        (const T*)mg.a, mg.lin_scale, mg.dr ? c->bwd_part_dr : nullptr);
-    LA_CUDA(c, cudaGetLastError());
+    LA_CUDA(c, (launch_chained(q_kernel, (unsigned)rb.P, threads, rb.small ? simt_bwd_smem<D, 1, true>() : simt_bwd_smem<D, 4, true>(), st, (const T*)q, (const T*)dout, c->Wq, c->state, (T*)dq, c->bwd_part_state, c->bwd_part_w, c->H, n, rb.Tn, rb.tiles, as, relu, (const T*)mg.a, mg.lin_scale, mg.dr ? c->bwd_part_dr : nullptr)));
     prof_mark(c, st, "qside_bwd", 3.0 * tensor_bytes);
     int launches = 5;
-    launch_combine_state<D>(rb, c->bwd_part_state, c->bwd_dstate, G, st);
-    LA_CUDA(c, cudaGetLastError());
+    LA_CUDA(c, (launch_combine_state<D>(rb, c->bwd_part_state, c->bwd_dstate, G, st)));
     const dim3 wgrid(DM / 256, per_head ? (unsigned)c->H : 1u);
     if (!relu) {   // the ReLU kernel function has no weights
-        combine_wgrad<<<wgrid, 512, 0, st>>>(c->bwd_part_w, dWq, (int)G, c->H, DM, per_head, rb.Tn, rb.tiles, rb.P);
-        LA_CUDA(c, cudaGetLastError());
+        LA_CUDA(c, (launch_chained(combine_wgrad, wgrid, 512, 0, st, c->bwd_part_w, dWq, (int)G, c->H, DM, per_head, rb.Tn, rb.tiles, rb.P)));
         ++launches;
     }
     if (mg.dr) {
-        combine_dr<<<1, 32, 0, st>>>(c->bwd_part_dr, (int)rb.P, mg.r_in_range, mg.dr);
-        LA_CUDA(c, cudaGetLastError());
+        LA_CUDA(c, (launch_chained(combine_dr, 1, 32, 0, st, c->bwd_part_dr, (int)rb.P, mg.r_in_range, mg.dr)));
         ++launches;
     }
     prof_mark(c, st, "combine_dstate_dWq", 0.0);
-    k_kernel<<<(unsigned)rb.P, threads, rb.small ? simt_bwd_smem<D, 1, false>() : simt_bwd_smem<D, 4, false>(), st>>>(
-        (const T*)k, (const T*)v, c->Wk, c->bwd_dstate, (T*)dk, (T*)dv, c->bwd_part_w, c->H, n, rb.Tn, rb.tiles, as, relu);
-    LA_CUDA(c, cudaGetLastError());
+    LA_CUDA(c, (launch_chained(k_kernel, (unsigned)rb.P, threads, rb.small ? simt_bwd_smem<D, 1, false>() : simt_bwd_smem<D, 4, false>(), st, (const T*)k, (const T*)v, c->Wk, c->bwd_dstate, (T*)dk, (T*)dv, c->bwd_part_w, c->H, n, rb.Tn, rb.tiles, as, relu)));
     prof_mark(c, st, "kside_bwd", 4.0 * tensor_bytes);
     if (!relu) {
-        combine_wgrad<<<wgrid, 512, 0, st>>>(c->bwd_part_w, dWk, (int)G, c->H, DM, per_head, rb.Tn, rb.tiles, rb.P);
-        LA_CUDA(c, cudaGetLastError());
+        LA_CUDA(c, (launch_chained(combine_wgrad, wgrid, 512, 0, st, c->bwd_part_w, dWk, (int)G, c->H, DM, per_head, rb.Tn, rb.tiles, rb.P)));
         ++launches;
     }
     prof_mark(c, st, "combine_dWk", 0.0);
@@ -449,13 +435,10 @@ linattn_status launch_tc(linattn_ctx* c, const void* q, const void* k, const voi
     }
     {
         void* kp[] = {&tmK, &tmV, &tmWk, &tmWklo, &a};
-        LA_CUDA(c, cudaLaunchKernel(k_kside[layout][phi][pair][split], dim3((unsigned)Pk), dim3(kThreads), kp, Smem::kTotal, st));
+        LA_CUDA(c, launch_chained_ptr(k_kside[layout][phi][pair][split], dim3((unsigned)Pk), dim3(kThreads), kp, Smem::kTotal, st));
     }
-    LA_CUDA(c, cudaGetLastError());
     prof_mark(c, st, "kside_tc", side_bytes);
-    if (pair) combine_tc<1><<<dim3((kE / 4 + 255) / 256, (unsigned)G), 256, 0, st>>>(a, Pk);
-    else combine_tc<0><<<dim3((kE / 4 + 255) / 256, (unsigned)G), 256, 0, st>>>(a, Pk);
-    LA_CUDA(c, cudaGetLastError());
+    LA_CUDA(c, launch_chained(pair ? combine_tc<1> : combine_tc<0>, dim3((kE / 4 + 255) / 256, (unsigned)G), 256, 0, st, a, Pk));
     prof_mark(c, st, "combine_tc", 0.0);
     if (state_only) {   // the backward pass wants S and z only
         c->last_launches = 2;
@@ -463,9 +446,8 @@ linattn_status launch_tc(linattn_ctx* c, const void* q, const void* k, const voi
     }
     {
         void* qp[] = {&tmQ, &tmO, &tmWq, &tmWqlo, &tmS, &tmA, &a};
-        LA_CUDA(c, cudaLaunchKernel(k_qside[mix ? 1 : 0][layout][phi][pair][split], dim3((unsigned)Pq), dim3(kThreads), qp, Smem::kTotal, st));
+        LA_CUDA(c, launch_chained_ptr(k_qside[mix ? 1 : 0][layout][phi][pair][split], dim3((unsigned)Pq), dim3(kThreads), qp, Smem::kTotal, st));
     }
-    LA_CUDA(c, cudaGetLastError());
     prof_mark(c, st, "qside_tc", side_bytes);
     c->last_launches = 3;
     return LINATTN_OK;
@@ -553,35 +535,30 @@ linattn_status launch_backward_tc(linattn_ctx* c, const void* q, const void* k, 
 #endif
     const dim3 wgrid(kWRec / 256, per_head ? (unsigned)c->H : 1u);
     if (need_lo) {   // the state was taken over from a forward that ran before the backward's workspace existed
-        hilo_images<<<dim3(kD * kD / 256, (unsigned)G), 256, 0, st>>>(c->state, nullptr, c->bwd_img[0]);
-        LA_CUDA(c, cudaGetLastError());
+        LA_CUDA(c, (launch_chained(hilo_images, dim3(kD * kD / 256, (unsigned)G), 256, 0, st, c->state, nullptr, c->bwd_img[0])));
         c->state_key.has_lo = true;
         ++launches;
     }
     {
         void* p[] = {&tmQ, &tmG, &tmDQ, &tmWq, &tmShi, &tmSlo, &a};
-        LA_CUDA(c, cudaLaunchKernel(k_q[layout][mg.dr ? 1 : 0], dim3((unsigned)P), dim3(kBwdThreads), p, kBwdSmemQ, st));
+        LA_CUDA(c, launch_chained_ptr(k_q[layout][mg.dr ? 1 : 0], dim3((unsigned)P), dim3(kBwdThreads), p, kBwdSmemQ, st));
     }
     prof_mark(c, st, "qside_bwd_tc", (mg.dr ? 4.0 : 3.0) * tensor_bytes);
     if (mg.dr) {
-        combine_dr<<<1, 32, 0, st>>>(c->bwd_part_dr, (int)P, mg.r_in_range, mg.dr);
-        LA_CUDA(c, cudaGetLastError());
+        LA_CUDA(c, (launch_chained(combine_dr, 1, 32, 0, st, c->bwd_part_dr, (int)P, mg.r_in_range, mg.dr)));
         ++launches;
     }
-    combine_slots_hilo<<<dim3((kE + 255) / 256, (unsigned)G), 256, 0, st>>>(c->bwd_part_state, c->bwd_dstate, c->bwd_img[1], c->bwd_img[2],
-                                                                           (int)Tn, T, P);
-    LA_CUDA(c, cudaGetLastError());
+    LA_CUDA(c, (launch_chained(combine_slots_hilo, dim3((kE + 255) / 256, (unsigned)G), 256, 0, st, c->bwd_part_state, c->bwd_dstate, c->bwd_img[1], c->bwd_img[2], (int)Tn, T, P)));
     prof_mark(c, st, "combine_dstate", 0.0);
     a.state = c->bwd_dstate;
     a.test_unmet = c->opt_unmet == 3 ? 1 : 0;
     a.part_w = c->bwd_part_w2;   // dW_k's records; dW_q's stay in part_w until both are summed at the end
     {
         void* p[] = {&tmK, &tmV, &tmDK, &tmDV, &tmWk, &tmDShi, &tmDSlo, &a};
-        LA_CUDA(c, cudaLaunchKernel(k_k[layout], dim3((unsigned)P), dim3(kBwdThreads), p, kBwdSmemK, st));
+        LA_CUDA(c, launch_chained_ptr(k_k[layout], dim3((unsigned)P), dim3(kBwdThreads), p, kBwdSmemK, st));
     }
     prof_mark(c, st, "kside_bwd_tc", 4.0 * tensor_bytes);
-    combine_wgrad_slots2<<<dim3(wgrid.x, wgrid.y, 2), 256, 0, st>>>(c->bwd_part_w, c->bwd_part_w2, dWq, dWk, (int)G, c->H, per_head, (int)Tn, T, P);
-    LA_CUDA(c, cudaGetLastError());
+    LA_CUDA(c, (launch_chained(combine_wgrad_slots2, dim3(wgrid.x, wgrid.y, 2), 256, 0, st, c->bwd_part_w, c->bwd_part_w2, dWq, dWk, (int)G, c->H, per_head, (int)Tn, T, P)));
     prof_mark(c, st, "combine_dWq_dWk", 0.0);
     c->last_launches = launches;
     return LINATTN_OK;
@@ -668,14 +645,14 @@ linattn_status launch_backward_split(linattn_ctx* c, const void* q, const void* 
     const double tensor_bytes = (double)heads * n * c->d * 2;
     const dim3 grid((unsigned)P), block(kSpThreads), cgrid((kE + 255) / 256, (unsigned)units);
     const dim3 wgrid((unsigned)(c->d * c->d / 2 + 255) / 256, per_head ? (unsigned)c->H : 1u);
+    // (plain launches: as a chain, see launch.cuh, these seven were 1 % slower, 366.6 against 362.8 us and 479.6 against 472.3 us)
     auto combine = [&](const float* rec, float* state) {
-        if (pair) combine_split<1><<<cgrid, 256, 0, st>>>(rec, c->bwd_img[0], c->bwd_img[1], c->bwd_img[2], c->bwd_vec, state, (int)heads, (int)Tn, T, P);
-        else combine_split<0><<<cgrid, 256, 0, st>>>(rec, c->bwd_img[0], c->bwd_img[1], c->bwd_img[2], c->bwd_vec, state, (int)heads, (int)Tn, T, P);
+        (pair ? combine_split<1> : combine_split<0>)<<<cgrid, 256, 0, st>>>(rec, c->bwd_img[0], c->bwd_img[1], c->bwd_img[2], c->bwd_vec, state,
+                                                                          (int)heads, (int)Tn, T, P);
         return cudaGetLastError();
     };
     auto combine_w = [&](float* dW) {
-        if (pair) combine_wgrad_split<1><<<wgrid, 256, 0, st>>>(c->bwd_part_w, dW, (int)heads, c->H, per_head, (int)Tn, T, P);
-        else combine_wgrad_split<0><<<wgrid, 256, 0, st>>>(c->bwd_part_w, dW, (int)heads, c->H, per_head, (int)Tn, T, P);
+        (pair ? combine_wgrad_split<1> : combine_wgrad_split<0>)<<<wgrid, 256, 0, st>>>(c->bwd_part_w, dW, (int)heads, c->H, per_head, (int)Tn, T, P);
         return cudaGetLastError();
     };
     int launches = 7;
@@ -695,8 +672,7 @@ linattn_status launch_backward_split(linattn_ctx* c, const void* q, const void* 
     }
     prof_mark(c, st, "qside_bwd_split_tc", (mg.dr ? 4.0 : 3.0) * tensor_bytes);
     if (mg.dr) {
-        combine_dr<<<1, 32, 0, st>>>(c->bwd_part_dr, (int)P, mg.r_in_range, mg.dr);
-        LA_CUDA(c, cudaGetLastError());
+        LA_CUDA(c, (launch_chained(combine_dr, 1, 32, 0, st, c->bwd_part_dr, (int)P, mg.r_in_range, mg.dr)));
         ++launches;
     }
     LA_CUDA(c, combine(c->bwd_part_state, nullptr));
@@ -1024,9 +1000,8 @@ static linattn_status backward_impl(linattn_ctx* c, const void* q, const void* k
     if (a && d_a) {
         const size_t count = (size_t)B * H * n * d;
         const unsigned blocks = (unsigned)((count + 256 * 8 - 1) / (256 * 8) < 1184 * 4 ? (count + 256 * 8 - 1) / (256 * 8) : 1184 * 4);
-        if (dtype == LINATTN_BF16) scale_copy<__nv_bfloat16><<<blocks, 256, 0, st>>>((const __nv_bfloat16*)dout, (__nv_bfloat16*)d_a, count, 1.f - mg.lin_scale);
-        else scale_copy<float><<<blocks, 256, 0, st>>>((const float*)dout, (float*)d_a, count, 1.f - mg.lin_scale);
-        LA_CUDA(c, cudaGetLastError());
+        if (dtype == LINATTN_BF16) LA_CUDA(c, launch_chained(scale_copy<__nv_bfloat16>, blocks, 256, 0, st, (const __nv_bfloat16*)dout, (__nv_bfloat16*)d_a, count, 1.f - mg.lin_scale));
+        else LA_CUDA(c, launch_chained(scale_copy<float>, blocks, 256, 0, st, (const float*)dout, (float*)d_a, count, 1.f - mg.lin_scale));
     }
     // bf16 activations with Eq. 6 run on the tensor cores: d = 128 with bf16 weights on the kernels with bf16 operands, d = 64
     // and fp32 weights on those that keep fp32 accuracy (if there is enough work); everything else on the CUDA cores

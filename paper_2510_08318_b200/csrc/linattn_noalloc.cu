@@ -82,10 +82,13 @@ linattn_status run(int dev, int slot, float* scratch, const T* q, const T* k, co
     float* state = scratch + (size_t)kNoAllocPartialSlots * kNoAllocMaxE;  // [G][E], fully overwritten
     const ActStrides as{D, (long long)n * D, (long long)Hw * n * D};
     const SimtRuns r = kside_runs<D>(G, n, (int)splits);
-    launch_kside_simt<T, D>(r, k, v, Wk, partial, Hw, n, as, 0, st);
-    launch_combine_state<D>(r, partial, state, G, st);
-    launch_qside_simt<T, D>(qside_runs<D>(G, n), q, Wq, state, out, Hw, n, (const T*)nullptr, 0.f, as, 0, st);
-    if (cudaGetLastError() != cudaSuccess) return LINATTN_ERR_CUDA;
+    cudaError_t e = launch_kside_simt<T, D>(r, k, v, Wk, partial, Hw, n, as, 0, st);
+    if (e == cudaSuccess) e = launch_combine_state<D>(r, partial, state, G, st);
+    if (e == cudaSuccess) e = launch_qside_simt<T, D>(qside_runs<D>(G, n), q, Wq, state, out, Hw, n, (const T*)nullptr, 0.f, as, 0, st);
+    if (e != cudaSuccess || cudaGetLastError() != cudaSuccess) {
+        cudaGetLastError();
+        return LINATTN_ERR_CUDA;
+    }
     return LINATTN_OK;
 }
 

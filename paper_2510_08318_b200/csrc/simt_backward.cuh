@@ -186,6 +186,8 @@ qside_bwd(const T* __restrict__ q, const T* __restrict__ dout, const float* __re
     using Ti = SimtTile<D, kSimtBwdWarps, TM>;
     constexpr int M = Sh::M, PX = Sh::PX, PW = Sh::PW, JG = Sh::JG, TG = Ti::TG, TT = Ti::TT, TH = Ti::kThreads;
     constexpr int NS = D * D / 64, SUB = TH / NS;
+    pdl_trigger();
+    pdl_wait();
     extern __shared__ __align__(16) float smem[];
     float* W_s = smem;
     float* S_s = W_s + D * PW;
@@ -324,6 +326,8 @@ kside_bwd(const T* __restrict__ k, const T* __restrict__ v, const float* __restr
     using Ti = SimtTile<D, kSimtBwdWarps, TM>;
     constexpr int M = Sh::M, PX = Sh::PX, PW = Sh::PW, JG = Sh::JG, TG = Ti::TG, TT = Ti::TT, TH = Ti::kThreads;
     constexpr int NS = D * D / 64, SUB = TH / NS;
+    pdl_trigger();
+    pdl_wait();
     extern __shared__ __align__(16) float smem[];
     float* W_s = smem;
     float* S_s = W_s + D * PW;
@@ -418,6 +422,8 @@ kside_bwd(const T* __restrict__ k, const T* __restrict__ v, const float* __restr
 static __global__ void __launch_bounds__(512)
 combine_wgrad(const float* __restrict__ rec, float* __restrict__ dW, int G, int H, int DM, int per_head, int Tn, long long tiles, long long P)
 {
+    pdl_trigger();
+    pdl_wait();
     __shared__ float4 part_s[8][64];
     const int lane = threadIdx.x & 63, slice = threadIdx.x >> 6;
     const int e = (blockIdx.x * 64 + lane) * 4, w = blockIdx.y, step = per_head ? H : 1;
@@ -457,6 +463,8 @@ combine_wgrad(const float* __restrict__ rec, float* __restrict__ dW, int G, int 
 // clip passes the gradient on the closed interval), else 0.  One warp.
 static __global__ void __launch_bounds__(32) combine_dr(const float* __restrict__ part_dr, int count, int in_range, float* __restrict__ dr)
 {
+    pdl_trigger();
+    pdl_wait();
     float acc = 0.f;
     for (int i = threadIdx.x; i < count; i += 32) acc += part_dr[i];
     acc = group_sum<32>(acc);
@@ -490,6 +498,8 @@ template <typename T, int D> cudaError_t simt_backward_attributes()
 template <typename T>
 static __global__ void __launch_bounds__(256) scale_copy(const T* __restrict__ src, T* __restrict__ dst, size_t count, float f)
 {
+    pdl_trigger();
+    pdl_wait();
     for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < count; i += (size_t)gridDim.x * 256) store_out(&dst[i], f * to_f32(src[i]));
 }
 

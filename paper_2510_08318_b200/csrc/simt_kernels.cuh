@@ -25,6 +25,7 @@
 #include <stdint.h>
 
 #include "f32x2.cuh"
+#include "launch.cuh"
 
 namespace linattn {
 
@@ -319,6 +320,8 @@ kside_simt(const T* __restrict__ k, const T* __restrict__ v, const float* __rest
     using Ti = SimtTile<D, kSimtKWarps, TM>;
     constexpr int TG = Ti::TG, TT = Ti::TT, PX = Sh::PX, JG = Sh::JG, TH = Ti::kThreads;
     constexpr int NS = D * D / 64, SUB = TH / NS;
+    pdl_trigger();
+    pdl_wait();
     extern __shared__ __align__(16) float smem[];
     float* W_s = smem;
     float* x_s = W_s + D * Sh::PW;
@@ -369,6 +372,8 @@ kside_simt(const T* __restrict__ k, const T* __restrict__ v, const float* __rest
 static __global__ void __launch_bounds__(256)
 combine_state(const float* __restrict__ rec, float* __restrict__ out, int E, int Tn, long long tiles, long long P, int slot_step)
 {
+    pdl_trigger();
+    pdl_wait();
     __shared__ float4 part_s[4][64];
     const int lane = threadIdx.x & 63, slice = threadIdx.x >> 6;
     const int e = (blockIdx.x * 64 + lane) * 4, g = blockIdx.y;
@@ -419,6 +424,8 @@ qside_simt(const T* __restrict__ q, const float* __restrict__ Wq, const float* _
     using Sh = SimtShape<D>;
     using Ti = SimtTile<D, NW, TM>;
     constexpr int TG = Ti::TG, TT = Ti::TT, PX = Sh::PX, JG = Sh::JG, TH = Ti::kThreads, M = Sh::M;
+    pdl_trigger();
+    pdl_wait();
     extern __shared__ __align__(16) float smem[];
     float* W_s = smem;
     float* S_s = W_s + D * Sh::PW;
@@ -549,27 +556,25 @@ template <typename T, int D> cudaError_t simt_forward_attributes()
 }
 
 template <typename T, int D>
-void launch_kside_simt(const SimtRuns& r, const T* k, const T* v, const float* Wk, float* partial, int H, int n, ActStrides st,
-                       int relu, cudaStream_t stream)
+cudaError_t launch_kside_simt(const SimtRuns& r, const T* k, const T* v, const float* Wk, float* partial, int H, int n, ActStrides st, int relu,
+                              cudaStream_t stream)
 {
-    if (r.small)
-        kside_simt<T, D, 1><<<(unsigned)r.P, 32 * kSimtKWarps, kside_simt_smem<D, 1>(), stream>>>(k, v, Wk, partial, H, n, r.Tn, r.tiles, r.slot_step, st, relu);
-    else
-        kside_simt<T, D, 4><<<(unsigned)r.P, 32 * kSimtKWarps, kside_simt_smem<D, 4>(), stream>>>(k, v, Wk, partial, H, n, r.Tn, r.tiles, r.slot_step, st, relu);
+    return launch_chained(r.small ? kside_simt<T, D, 1> : kside_simt<T, D, 4>, (unsigned)r.P, 32 * kSimtKWarps,
+                          r.small ? kside_simt_smem<D, 1>() : kside_simt_smem<D, 4>(), stream, k, v, Wk, partial, H, n, r.Tn, r.tiles, r.slot_step,
+                          st, relu);
 }
-template <int D> void launch_combine_state(const SimtRuns& r, const float* partial, float* state, long long G, cudaStream_t stream)
+template <int D> cudaError_t launch_combine_state(const SimtRuns& r, const float* partial, float* state, long long G, cudaStream_t stream)
 {
     constexpr int E = SimtShape<D>::E;
-    combine_state<<<dim3((E + 255) / 256, (unsigned)G), 256, 0, stream>>>(partial, state, E, r.Tn, r.tiles, r.P, r.slot_step);
+    return launch_chained(combine_state, dim3((E + 255) / 256, (unsigned)G), 256, 0, stream, partial, state, E, r.Tn, r.tiles, r.P, r.slot_step);
 }
 template <typename T, int D>
-void launch_qside_simt(const SimtRuns& r, const T* q, const float* Wq, const float* state, T* out, int H, int n, const T* mix, float mix_r,
-                       ActStrides st, int relu, cudaStream_t stream)
+cudaError_t launch_qside_simt(const SimtRuns& r, const T* q, const float* Wq, const float* state, T* out, int H, int n, const T* mix, float mix_r,
+                              ActStrides st, int relu, cudaStream_t stream)
 {
-    if (r.small)
-        qside_simt<T, D, 8, 1><<<(unsigned)r.P, 256, qside_simt_smem<D, 8, 1>(), stream>>>(q, Wq, state, out, H, n, r.Tn, r.tiles, mix, mix_r, st, relu);
-    else
-        qside_simt<T, D, kSimtQWarps, 4><<<(unsigned)r.P, 32 * kSimtQWarps, qside_simt_smem<D, kSimtQWarps, 4>(), stream>>>(q, Wq, state, out, H, n, r.Tn, r.tiles, mix, mix_r, st, relu);
+    return launch_chained(r.small ? qside_simt<T, D, 8, 1> : qside_simt<T, D, kSimtQWarps, 4>, (unsigned)r.P, r.small ? 256 : 32 * kSimtQWarps,
+                          r.small ? qside_simt_smem<D, 8, 1>() : qside_simt_smem<D, kSimtQWarps, 4>(), stream, q, Wq, state, out, H, n, r.Tn,
+                          r.tiles, mix, mix_r, st, relu);
 }
 
 // Feature-map weights: any supported storage type -> fp32 [H][D][M]; src is [H][D][M] or, when per_head == 0, a single

@@ -153,12 +153,14 @@ __device__ __forceinline__ bool bwd_smem_fits(const uint8_t* smem_raw, uint32_t 
     asm volatile("mov.u32 %0, %%dynamic_smem_size;" : "=r"(have));
     const uint32_t pad = (1024u - (smem_u32(smem_raw) & 1023u)) & 1023u;
     if (pad + need <= have) return true;
+    pdl_wait();
     if (threadIdx.x == 0) atomicOr(err, kErrSmem);
     return false;
 }
 
 __device__ __forceinline__ BwdCta bwd_setup(uint8_t* smem_raw, uint32_t misc_off, uint32_t* err, uint32_t wait_limit_us)
 {
+    pdl_trigger();
     BwdCta c;
     c.smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     c.sbase = smem_u32(c.smem);
@@ -179,6 +181,7 @@ __device__ __forceinline__ BwdCta bwd_setup(uint8_t* smem_raw, uint32_t misc_off
         tmem_alloc(smem_u32(tmem_slot), 512);
         tmem_relinquish();
     }
+    pdl_wait();
     fence_proxy_async_smem();
     tcgen05_fence_before();
     __syncthreads();
@@ -1094,26 +1097,14 @@ kside_bwd_tc(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
     bwd_teardown(c);
 }
 
-// out[g][e] = sum over the CTAs that own tiles of head g, ascending, of part[(cta + g)][e].  grid = (ceil(E/256), G).
-static __global__ void __launch_bounds__(256)
-combine_slots(const float* __restrict__ part, float* __restrict__ out, int E, int tiles_per_head, long long total_tiles, long long P)
-{
-    const int e = blockIdx.x * 256 + threadIdx.x;
-    if (e >= E) return;
-    const int g = blockIdx.y;
-    const long long c0 = tile_owner((long long)g * tiles_per_head, total_tiles, P);
-    const long long c1 = tile_owner((long long)(g + 1) * tiles_per_head - 1, total_tiles, P);
-    float acc = 0.f;
-    for (long long cta = c0; cta <= c1; ++cta) acc += part[(size_t)(cta + g) * E + e];
-    out[(size_t)g * E + e] = acc;
-}
-
-// The two steps in one for dS, dz: fixed-order sum of the (CTA, head) records, fp32 state and, for the matrix part, the
+// dS, dz: fixed-order sum of the (CTA, head) records (over the CTAs that own tiles of head g, ascending), fp32 state and, for the matrix part, the
 // bf16 hi and lo images the key side reads.  grid = (ceil(kE/256), G).
 static __global__ void __launch_bounds__(256)
 combine_slots_hilo(const float* __restrict__ part, float* __restrict__ out, __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo,
                    int tiles_per_head, long long total_tiles, long long P)
 {
+    pdl_trigger();
+    pdl_wait();
     const int e = blockIdx.x * 256 + threadIdx.x;
     if (e >= kE) return;
     const int g = blockIdx.y;
@@ -1133,6 +1124,8 @@ combine_slots_hilo(const float* __restrict__ part, float* __restrict__ out, __nv
 static __global__ void __launch_bounds__(256)
 hilo_images(const float* __restrict__ state, __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo)
 {
+    pdl_trigger();
+    pdl_wait();
     const int e = blockIdx.x * 256 + threadIdx.x, g = blockIdx.y;
     const float x = state[(size_t)g * kE + e];
     const __nv_bfloat16 h = __float2bfloat16_rn(x);
@@ -1141,27 +1134,14 @@ hilo_images(const float* __restrict__ state, __nv_bfloat16* __restrict__ hi, __n
 }
 
 // dW[w][c][j] = sum over the heads g that use weight matrix w (per_head: g % H == w; shared: all), ascending, and
-// over the CTAs of each, ascending, of part_w[(cta + g)][j][c].  grid = (kWRec / 256, per_head ? H : 1).
-static __global__ void __launch_bounds__(256)
-combine_wgrad_slots(const float* __restrict__ part_w, float* __restrict__ dW, int G, int H, int per_head, int tiles_per_head,
-                    long long total_tiles, long long P)
-{
-    const int r = blockIdx.x * 256 + threadIdx.x;   // index in a record, j * 128 + c: neighbouring threads read neighbouring words
-    const int j = r / kD, cc = r % kD, wsel = blockIdx.y;
-    float acc = 0.f;
-    for (int g = per_head ? wsel : 0; g < G; g += per_head ? H : 1) {
-        const long long c0 = tile_owner((long long)g * tiles_per_head, total_tiles, P);
-        const long long c1 = tile_owner((long long)(g + 1) * tiles_per_head - 1, total_tiles, P);
-        for (long long cta = c0; cta <= c1; ++cta) acc += part_w[(size_t)(cta + g) * kWRec + r];
-    }
-    dW[(size_t)wsel * kWRec + (size_t)cc * kM + j] = acc;
-}
-
+// over the CTAs of each, ascending, of part_w[(cta + g)][j][c].
 // Both weight gradients in one launch: blockIdx.z = 0: dW_q from part_wq, 1: dW_k from part_wk.  grid = (kWRec / 256, per_head ? H : 1, 2).
 static __global__ void __launch_bounds__(256)
 combine_wgrad_slots2(const float* __restrict__ part_wq, const float* __restrict__ part_wk, float* __restrict__ dWq, float* __restrict__ dWk,
                      int G, int H, int per_head, int tiles_per_head, long long total_tiles, long long P)
 {
+    pdl_trigger();
+    pdl_wait();
     const float* part_w = blockIdx.z == 0 ? part_wq : part_wk;
     float* dW = blockIdx.z == 0 ? dWq : dWk;
     const int r = blockIdx.x * 256 + threadIdx.x;

@@ -32,6 +32,7 @@
 #include <stdint.h>
 
 #include "f32x2.cuh"
+#include "launch.cuh"
 #include "sm100_ptx.cuh"
 
 namespace linattn {
@@ -413,6 +414,7 @@ struct Args {
 // Common prologue: barrier init, TMEM allocation (512 columns, warp 9), abort word.
 __device__ __forceinline__ Cta cta_setup(uint8_t* smem_raw, const Args& a, bool init_k, bool init_q)
 {
+    pdl_trigger();
     Cta c;
     c.smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     c.sbase = smem_u32(c.smem);
@@ -450,6 +452,7 @@ __device__ __forceinline__ Cta cta_setup(uint8_t* smem_raw, const Args& a, bool 
     }
     if (init_k)
         for (int i = threadIdx.x; i < 512; i += blockDim.x) reinterpret_cast<__nv_bfloat16*>(c.smem + Smem::kOnes)[i] = __float2bfloat16(1.0f);
+    pdl_wait();
     fence_proxy_async_smem();
     tcgen05_fence_before();
     __syncthreads();
@@ -1259,6 +1262,8 @@ kside_tc(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtens
 template <int kPair>
 __global__ void __launch_bounds__(256) combine_tc(const Args a, long long P)
 {
+    pdl_trigger();
+    pdl_wait();
     const int q4 = blockIdx.x * 256 + threadIdx.x;
     if (q4 < kE / 4) combine_quad<kPair>(a, P, blockIdx.y, q4 * 4);
 }

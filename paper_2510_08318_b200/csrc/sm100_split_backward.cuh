@@ -102,6 +102,7 @@ struct SpCta {
 
 __device__ __forceinline__ SpCta sp_setup(uint8_t* raw, uint32_t misc_off, uint32_t* err, uint32_t limit_us)
 {
+    pdl_trigger();
     SpCta c;
     c.smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
     c.sb = smem_u32(c.smem);
@@ -121,6 +122,7 @@ __device__ __forceinline__ SpCta sp_setup(uint8_t* raw, uint32_t misc_off, uint3
         tmem_alloc(smem_u32(slot), 512);
         tmem_relinquish();
     }
+    pdl_wait();
     fence_proxy_async_smem();
     tcgen05_fence_before();
     __syncthreads();
@@ -964,6 +966,8 @@ static __global__ void __launch_bounds__(256)
 combine_split(const float* __restrict__ rec, __nv_bfloat16* __restrict__ img0, __nv_bfloat16* __restrict__ img1, __nv_bfloat16* __restrict__ img2,
               float* __restrict__ vec, float* __restrict__ state, int heads, int tiles_per_unit, long long total_tiles, long long P)
 {
+    pdl_trigger();
+    pdl_wait();
     __shared__ float4 part_s[4][64];
     const int lane = threadIdx.x & 63, slice = threadIdx.x >> 6;
     const int e = (blockIdx.x * 64 + lane) * 4, g = blockIdx.y;
@@ -1020,6 +1024,8 @@ static __global__ void __launch_bounds__(256)
 combine_wgrad_split(const float* __restrict__ rec, float* __restrict__ dW, int heads, int H, int per_head, int tiles_per_unit, long long total_tiles,
                     long long P)
 {
+    pdl_trigger();
+    pdl_wait();
     constexpr int d = kPair ? 64 : 128, m = d / 2;
     __shared__ float4 part_s[4][64];
     const int lane = threadIdx.x & 63, slice = threadIdx.x >> 6, wsel = blockIdx.y;
